@@ -644,9 +644,13 @@ __device__ __forceinline__ void res_env(const ResArgs& a, const RateView& kv, co
             if (tid == 0) T.n_list[(s + 1) & 1] = 0;
             __syncthreads();
             res_load(a.F0 + off, H, W, WW, vec, Bc, C, D, word_list(s + 1), dirty, 1, &T.burnt, tid, NT);
+            // the drop is read ahead of the barrier: thread 0 of the next step
+            // writes the following one over it, and a grid without a drop meets
+            // no further barrier before
+            const int cxn = T.drop[0], cyn = T.drop[1];
             __syncthreads();
-            if (T.drop[0] >= 0) {
-                res_action(H, W, WW, Bc, D, dirty, T.drop[0], T.drop[1], a.R, tid, NT, &T.burnt);
+            if (cxn >= 0) {
+                res_action(H, W, WW, Bc, D, dirty, cxn, cyn, a.R, tid, NT, &T.burnt);
                 __syncthreads();
             } else if (a.mask != nullptr && next_act) {
                 res_action_mask(a.mask + (int64_t)(s + 1) * a.mask_words, off, H, W, WW, Bc, D, dirty, tid, NT,
