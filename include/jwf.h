@@ -513,9 +513,7 @@ JWF_API jwf_status jwf_relaxed_bwd_steps(jwf_ctx* ctx, int32_t n_steps, const fl
                                          float* d_gburn, float* d_glam, double* d_gpc, void* stream);
 
 /* jwf_relaxed_bwd_steps and jwf_rates_accumulate of the same steps in one call,
- * with the rates kept on chip over the adjoint steps (the same results; the
- * terms of dL/dp_continue are added in the order of jwf_relaxed_bwd_steps with
- * column_order != 0 and in small batches, else more exactly):
+ * with the rates kept on chip over the adjoint steps (the same results):
  * d_gr (float [cells][8], 16-byte aligned) and d_gpc (double[1] or NULL) are
  * added to, d_scratch is float [2][n_steps][cells].  Only where
  * jwf_relaxed_on_chip(ctx, with_masks) is 1 (every grid's rates fit a
@@ -526,7 +524,7 @@ JWF_API jwf_status jwf_relaxed_bwd_rates(jwf_ctx* ctx, int32_t n_steps, const fl
                                          const float* d_pburn, const float* d_masks,
                                          const float* d_gun_out, const float* d_gburn_out, float* d_gun,
                                          float* d_gburn, float* d_scratch, float* d_gr, double* d_gpc,
-                                         int32_t column_order, void* stream);
+                                         void* stream);
 
 /* The two halves of jwf_rates_bwd, for a backward pass that contracts once:
  * jwf_rates_accumulate adds the rate adjoint of n_steps relaxed steps,

@@ -1012,7 +1012,7 @@ int32_t jwf_relaxed_on_chip(jwf_ctx* ctx, int32_t with_masks) {
 jwf_status jwf_relaxed_bwd_rates(jwf_ctx* ctx, int32_t n_steps, const float* d_pun, const float* d_pburn,
                                  const float* d_masks, const float* d_gun_out, const float* d_gburn_out,
                                  float* d_gun, float* d_gburn, float* d_scratch, float* d_gr, double* d_gpc,
-                                 int32_t column_order, void* stream) {
+                                 void* stream) {
     if (ctx == nullptr) return JWF_EINVAL;
     if (n_steps < 1) return fail(ctx, JWF_EINVAL, "jwf_relaxed_bwd_rates: n_steps < 1");
     if (d_pun == nullptr || d_pburn == nullptr || d_gun_out == nullptr || d_gburn_out == nullptr ||
@@ -1037,7 +1037,7 @@ jwf_status jwf_relaxed_bwd_rates(jwf_ctx* ctx, int32_t n_steps, const float* d_p
         return fail(ctx, JWF_EUNSUPPORTED, "jwf_relaxed_bwd_rates: the grids do not fit on chip");
     float* ab = d_scratch + nC;
     JWF_CUDA_TRY(ctx, jwf_launch_band_bwd(ctx, n_steps, d_pun, d_pburn, d_masks, d_gun_out, d_gburn_out, d_gun,
-                                          d_gburn, d_scratch, ab, &d_gpc, column_order != 0, S(stream)),
+                                          d_gburn, d_scratch, ab, S(stream)),
                  "jwf_relaxed_bwd_rates");
     JWF_CUDA_TRY(ctx, jwf_launch_rates_accumulate(ctx, n_steps, d_scratch, d_pburn, d_masks, d_gr, ab, d_gpc,
                                                   S(stream)),

@@ -103,7 +103,7 @@ _SIGS = {
     "jwf_relaxed_fwd_steps": (ctypes.c_int, [_VP, ctypes.c_int32] + [_VP] * 6),
     "jwf_relaxed_bwd_steps": (ctypes.c_int, [_VP, ctypes.c_int32] + [_VP] * 10),
     "jwf_relaxed_on_chip": (ctypes.c_int32, [_VP, ctypes.c_int32]),
-    "jwf_relaxed_bwd_rates": (ctypes.c_int, [_VP, ctypes.c_int32] + [_VP] * 10 + [ctypes.c_int32, _VP]),
+    "jwf_relaxed_bwd_rates": (ctypes.c_int, [_VP, ctypes.c_int32] + [_VP] * 11),
     "jwf_rates_contract": (ctypes.c_int, [_VP] * 8),
     "jwf_mask_words": (ctypes.c_int64, [ctypes.c_int64]),
     "jwf_pack_masks": (ctypes.c_int, [ctypes.c_int32, ctypes.c_int64, _VP, _VP, _VP]),
@@ -595,13 +595,12 @@ class Sim:
         return bool(lib().jwf_relaxed_on_chip(self._h, int(bool(with_masks))))
 
     def relaxed_bwd_rates(self, pun, pburn, gun_out, gburn_out, gun, gburn, scratch, gr, masks=None, gpc=None,
-                          column_order: bool = False, stream=None):
+                          stream=None):
         """relaxed_bwd_steps and rates_accumulate (into gr) of the n steps of pun / pburn; scratch [2 * n, cells]."""
         n = pun.shape[0]
         self._check(lib().jwf_relaxed_bwd_rates(self._h, int(n), _ptr(pun), _ptr(pburn), _ptr(masks), _ptr(gun_out),
                                                 _ptr(gburn_out), _ptr(gun), _ptr(gburn), _ptr(scratch), _ptr(gr),
-                                                _ptr(gpc), int(bool(column_order)), _stream(stream)),
-                    "jwf_relaxed_bwd_rates")
+                                                _ptr(gpc), _stream(stream)), "jwf_relaxed_bwd_rates")
         return gun, gburn
 
     def rates_bwd(self, glam, pburn, cls, dem, wind_speed, wind_dir, gparams, mask=None, stream=None):

@@ -60,12 +60,11 @@ def theta_to_params(theta: torch.Tensor, n_classes: int, cell_size: float = 30.0
                         mu_veg=np.array(v[6:6 + C], np.float32), mu_den=np.array(v[6 + C:6 + 2 * C], np.float32))
 
 
-def _adjoint_chunk(sim, su, sb, gu, gb, ngu, ngb, masks, scratch, gr, gpc, column_order=False):
+def _adjoint_chunk(sim, su, sb, gu, gb, ngu, ngb, masks, scratch, gr, gpc):
     """Adjoint of one block of steps, its rate adjoint added to gr; scratch [CHUNK or, on chip, 2 * CHUNK, cells]."""
     n = su.shape[0]
     if sim.relaxed_on_chip(masks is not None):
-        sim.relaxed_bwd_rates(su, sb, gu, gb, ngu, ngb, scratch[:2 * n], gr, masks=masks, gpc=gpc,
-                              column_order=column_order)
+        sim.relaxed_bwd_rates(su, sb, gu, gb, ngu, ngb, scratch[:2 * n], gr, masks=masks, gpc=gpc)
         return
     sim.relaxed_bwd_steps(su, sb, gu, gb, ngu, ngb, masks=masks, glam=scratch[:n], gpc=gpc)
     sim.rates_accumulate(scratch[:n], sb, gr, mask=masks)
@@ -222,7 +221,7 @@ class StraightThroughRollout(torch.autograd.Function):
         hi = T
         while hi > 0:
             lo = ((hi - 1) // CHUNK) * CHUNK
-            _adjoint_chunk(sim, PU[lo:hi], PB[lo:hi], gu, gb, ngu, ngb, None, scratch, gr, gpc, column_order=True)
+            _adjoint_chunk(sim, PU[lo:hi], PB[lo:hi], gu, gb, ngu, ngb, None, scratch, gr, gpc)
             gu, ngu = ngu, gu
             gb, ngb = ngb, gb
             hi = lo
