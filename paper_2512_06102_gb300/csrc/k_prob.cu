@@ -463,9 +463,14 @@ k_rates_accumulate(const int4* __restrict__ tiles, int64_t n_tiles, const int32_
             for (int k = 0; k < kAccCPT; ++k) {
                 const float c0 = c[(k + 1) * A::W - 1], c1 = c[(k + 1) * A::W], c2 = c[(k + 1) * A::W + 1];
                 const float src[8] = {b0, c0, c1, c2, b2, a2, a1, a0};
-                if ((__float_as_uint(b0) | __float_as_uint(c0) | __float_as_uint(c1) | __float_as_uint(c2) |
-                     __float_as_uint(b2) | __float_as_uint(a2) | __float_as_uint(a1) | __float_as_uint(a0)) != 0u) {
-                    const float g = b.gl[(ty * kAccCPT + k) * A::Cols + tx];
+                uint32_t bits = __float_as_uint(b0) | __float_as_uint(c0) | __float_as_uint(c1) | __float_as_uint(c2) |
+                                __float_as_uint(b2) | __float_as_uint(a2) | __float_as_uint(a1) | __float_as_uint(a0);
+                const float* gl = &b.gl[(ty * kAccCPT + k) * A::Cols + tx];
+                // (a caller's glam may be infinite or NaN, whose product with 0 is
+                // not 0; the on-chip adjoint's is saturated)
+                if constexpr (!GPC) bits |= (__float_as_uint(*gl) & 0x7f800000u) == 0x7f800000u ? 1u : 0u;
+                if (bits != 0u) {
+                    const float g = *gl;
 #pragma unroll
                     for (int d = 0; d < 8; ++d) w[k][d] += g * src[d];
                 }
