@@ -304,8 +304,10 @@ JWF_API jwf_status jwf_state_planes(jwf_ctx* ctx, int32_t n, const uint8_t* d_st
                                     float* d_pburn, void* stream);
 
 /* Kernel choice for jwf_step (default JWF_KERNEL_AUTO: resident when every
- * env fits shared memory, else tiled, else (auto-reset) plain).  All kernels
- * give identical results for the same probabilities. */
+ * env fits shared memory, else tiled, else (auto-reset) plain; fewer envs than
+ * SMs that nearly fill an SM's shared memory are tiled too, or plain in
+ * launches of one step with auto-reset).  All kernels give identical results
+ * for the same probabilities. */
 typedef enum {
     JWF_KERNEL_AUTO = 0,      /* resident when every env fits shared memory  */
     JWF_KERNEL_PLAIN = 1,     /* one launch per step, state in global memory */
@@ -316,8 +318,9 @@ typedef enum {
                                  the table; bit-identical to the table built
                                  by jwf_precompute_probs from that terrain;
                                  tiled (below) for envs too large for shared
-                                 memory                                      */
-    JWF_KERNEL_TILED = 4,     /* 128 x 256-cell tiles with a halo, up to 16
+                                 memory and, without auto-reset, for few envs
+                                 that nearly fill it                         */
+    JWF_KERNEL_TILED = 4,     /* 64 x 128-cell tiles with a halo, up to 16
                                  steps per launch (temporal blocking); tiles
                                  with no fire within reach are skipped; for
                                  grids larger than shared memory.  Without
@@ -325,9 +328,10 @@ typedef enum {
     JWF_KERNEL_TILED_FUSED = 5 /* tiled, probabilities from the terrain      */
 } jwf_kernel;
 /* Choose the step kernel; threads_per_env = 0 picks a block size by env size
- * (resident kernels) or 256 threads a tile (tiled kernels); else 32, 64, 128,
- * 256, 512 or 1024 threads per env (resident kernels) or 128, 256 or 512
- * threads a tile (tiled kernels).  Other values return JWF_EINVAL. */
+ * and number (resident kernels) or 512 threads a tile, with the table and more
+ * than 2048 tiles 256 (tiled kernels); else 32, 64, 128, 256, 512 or 1024
+ * threads per env (resident kernels) or 128, 256 or 512 threads a tile (tiled
+ * kernels).  Other values return JWF_EINVAL. */
 JWF_API jwf_status jwf_set_kernel(jwf_ctx* ctx, jwf_kernel kernel, int32_t threads_per_env);
 
 /* Resident envs run as up to four size classes by their longer side (<= 64,
@@ -335,10 +339,9 @@ JWF_API jwf_status jwf_set_kernel(jwf_ctx* ctx, jwf_kernel kernel, int32_t threa
  * side on forked streams.  jwf_size_classes writes the classes present to
  * h_classes (host, up to 4 entries, may be NULL) and returns their number;
  * jwf_set_class_threads sets the block size of one class (0: by size; 32,
- * 64, 128, 256, 512 or 1024), e.g. from an autotuner; a block size whose
- * shared memory (it grows with the warps) does not fit the class's largest env
- * returns JWF_EINVAL and changes nothing.  jwf_set_kernel's explicit
- * threads_per_env overrides both. */
+ * 64, 128, 256, 512 or 1024), e.g. from an autotuner; for a class whose
+ * largest env does not fit shared memory any returns JWF_EINVAL and changes
+ * nothing.  jwf_set_kernel's explicit threads_per_env overrides both. */
 JWF_API int32_t jwf_size_classes(const jwf_ctx* ctx, int32_t* h_classes);
 JWF_API jwf_status jwf_set_class_threads(jwf_ctx* ctx, int32_t size_class, int32_t threads);
 

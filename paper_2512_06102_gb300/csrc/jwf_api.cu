@@ -56,12 +56,21 @@ void free_all(jwf_ctx* c) {
 
 inline cudaStream_t S(void* stream) { return reinterpret_cast<cudaStream_t>(stream); }
 
-bool use_resident(const jwf_ctx* c) {
-    if (c->kernel == JWF_KERNEL_PLAIN) return false;
-    // the step's constants, and by default 16 KB for more than the least queue
-    // and lists: grids that leave less are stepped by tiles, on many SMs
-    const size_t extra = c->threads_per_env > 0 ? sizeof(RateConsts) : 16000;
-    return jwf_resident_smem(c->maxH, c->maxW) + extra + 64 <= (size_t)c->smem_optin;
+// The resident step can take the context's grids: the least that a launch
+// needs, with the rate constants of the fused variant.
+bool resident_fits(const jwf_ctx* c, bool fused) {
+    return jwf_resident_smem(c->maxH, c->maxW) + (fused ? sizeof(RateConsts) : 0) + 64 <= (size_t)c->smem_optin;
+}
+
+// Grids that fit but whose planes nearly fill an SM, and fewer of them than
+// SMs: tiles, which spread each over many SMs, are faster (617 x 641, 100 steps
+// fused, resident and tiled, us: 1 grid 992 and 793, 38 grids 1922 and 1027; 152
+// grids 1759 and 2227; with the table 38 grids 1252 and 1115, 152 1212 and 1636).
+// The line is where the warps' 2.3 KB each, which the resident step once took
+// beside the planes, ended; smaller grids were resident then too.
+bool few_large(const jwf_ctx* c) {
+    return c->N < c->num_sms &&
+           jwf_resident_smem_roomy(c->maxH, c->maxW, c->threads_per_env) > (size_t)c->smem_optin;
 }
 
 }  // namespace
@@ -590,13 +599,18 @@ jwf_status step_impl(jwf_ctx* ctx, int32_t k, const int32_t* d_drops, const uint
     const bool fused = kn == JWF_KERNEL_FUSED || kn == JWF_KERNEL_TILED_FUSED;
     if (fused && !ctx->have_terrain) return fail(ctx, JWF_ESTATE, "jwf_step: fused step needs jwf_set_terrain");
     if (!fused && !ctx->have_table) return fail(ctx, JWF_ESTATE, "jwf_step: no probability table");
-    const bool fits = use_resident(ctx);
+    const bool fits = resident_fits(ctx, fused);
     if (kn == JWF_KERNEL_RESIDENT && !fits)
         return fail(ctx, JWF_EUNSUPPORTED, "jwf_step: largest env does not fit shared memory");
-    bool tiled = kn == JWF_KERNEL_TILED || kn == JWF_KERNEL_TILED_FUSED ||
-                 ((kn == JWF_KERNEL_AUTO || kn == JWF_KERNEL_FUSED) && !fits);
-    bool plain = kn == JWF_KERNEL_PLAIN;
-    if (tiled && (ctx->flags & JWF_AUTO_RESET)) {
+    const bool reset = (ctx->flags & JWF_AUTO_RESET) != 0u;
+    const bool by_size = kn == JWF_KERNEL_AUTO || kn == JWF_KERNEL_FUSED;
+    const bool few = by_size && fits && few_large(ctx);
+    bool tiled = kn == JWF_KERNEL_TILED || kn == JWF_KERNEL_TILED_FUSED || (by_size && (!fits || (few && !reset)));
+    // (tiles cannot restart a grid; a launch of one step of few large grids is
+    // shorter on the plain kernel: 617 x 641, 40 such launches, 1080 and 1590 us,
+    // one of 100 steps 2793 and 510)
+    bool plain = kn == JWF_KERNEL_PLAIN || (kn == JWF_KERNEL_AUTO && few && reset && k == 1);
+    if (tiled && reset) {
         // rounds of several steps cannot restart an env part-way: one launch per step
         if (fused) return fail(ctx, JWF_EUNSUPPORTED, "jwf_step: auto-reset on large grids needs the table");
         tiled = false;
@@ -770,7 +784,7 @@ jwf_status jwf_set_class_threads(jwf_ctx* ctx, int32_t size_class, int32_t threa
         return fail(ctx, JWF_EINVAL, "jwf_set_class_threads: threads must be 0, 32, 64, 128, 256, 512 or 1024");
     for (const JwfGroup& G : ctx->groups)
         if (G.size_class == size_class && threads > 0 &&
-            jwf_resident_smem(G.maxH, G.maxW) + sizeof(RateConsts) + 64 > (size_t)ctx->smem_optin)
+            jwf_resident_smem(G.maxH, G.maxW) + 64 > (size_t)ctx->smem_optin)
             return fail(ctx, JWF_EINVAL, "jwf_set_class_threads: the class's envs and that block size do not fit "
                                          "shared memory");
     for (JwfGroup& G : ctx->groups)

@@ -390,8 +390,11 @@ cudaError_t jwf_launch_pack_masks(int32_t n_rows, int64_t cells, const uint8_t* 
 cudaError_t jwf_build_tile_maps(jwf_ctx* c);
 int jwf_tile_rows();
 int jwf_tile_cols();
-// least shared memory a resident launch needs for env shape (H, W)
+// least shared memory a resident launch needs for env shape (H, W), without the
+// fused variant's constants; and with room for `threads` threads (0: 256), by
+// which few large grids go to tiles
 size_t jwf_resident_smem(int32_t H, int32_t W);
+size_t jwf_resident_smem_roomy(int32_t H, int32_t W, int32_t threads);
 
 // two relaxed steps in one pass (tiled kernels only): the state after step t
 // (pun1, pburn1) and after step t + 1 (pun2, pburn2); masks of the two steps

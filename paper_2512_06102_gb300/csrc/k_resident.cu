@@ -791,6 +791,13 @@ static size_t res_smem(int32_t H, int32_t W, int qcap, int lcap) {
 // the least a launch needs: what decides whether a shape is stepped here
 size_t jwf_resident_smem(int32_t H, int32_t W) { return res_smem(H, W, kResQMin, kResLMin); }
 
+// planes, 6 B a chunk of 32 words, 4.2 KB, 2.3 KB a warp
+size_t jwf_resident_smem_roomy(int32_t H, int32_t W, int32_t threads) {
+    const size_t chunks = ((size_t)H * ((W + 31) / 32) + 31) / 32;
+    return sizeof(uint32_t) * ((size_t)res_plane_words(H, W) + chunks + 2 * ((chunks + 3) / 4)) + 4256 +
+           2304 * (size_t)((threads > 0 ? threads : 256) / 32);
+}
+
 // Capacities of the work queue and of the lists of active words: eight items a
 // word (a front crosses a word's 32 cells with a handful of burning cells and
 // up to eight pairs each) and every word, as far as the CTAs that share an SM
