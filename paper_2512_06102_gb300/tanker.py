@@ -37,6 +37,16 @@ class TankerEnv:
         return self.obs, self.reward, self.done
 
 
+# the functions that jwf_agent_rollout stands for (a replaced one is another)
+_ENV_STEP, _SIM_STEP = TankerEnv.step, jwf.Sim.agent_step
+
+
+def _own_steps(env) -> bool:
+    """The env's step is TankerEnv's and its simulator's agent step is Sim's: neither a subclass's nor a replaced one."""
+    return (getattr(env.step, "__func__", None) is _ENV_STEP
+            and getattr(env.sim.agent_step, "__func__", None) is _SIM_STEP)
+
+
 class GraphTankerRollout:
     """T agent steps with actions[t] (int32 [T, N], device) as one CUDA graph;
     rewards and done flags are recorded as [T, N].  Capturing runs one
@@ -59,8 +69,8 @@ class GraphTankerRollout:
 
     def _body(self, T: int):
         env = self.env
-        if T > 0 and type(env).step is TankerEnv.step:
-            # all the steps in one call (an env with its own step goes step by step)
+        if T > 0 and _own_steps(env):
+            # all the steps in one call (an env or a simulator with its own step goes step by step)
             env.sim.agent_rollout(self.actions[:T], env.agent, env.water0, env.random_fire, env.burn_penalty,
                                   self.rewards[:T], self.dones[:T], env.obs_k, env.obs)
             env.reward.copy_(self.rewards[T - 1])
