@@ -461,8 +461,18 @@ cudaError_t jwf_launch_agent_warp(const jwf_ctx* c, bool fused, int32_t T, const
     a.burn_penalty = burn_penalty;
     const RateConsts& K = c->K;
     const unsigned grid = (unsigned)((c->N + kAgentWarps - 1) / kAgentWarps);
-    auto k = T > 1 ? (fused ? k_agent_warp<true, true> : k_agent_warp<false, true>)
-                   : (fused ? k_agent_warp<true, false> : k_agent_warp<false, false>);
+    auto one = fused ? k_agent_warp<true, false> : k_agent_warp<false, false>;
+    auto many = fused ? k_agent_warp<true, true> : k_agent_warp<false, true>;
+    auto k = T > 1 ? many : one;
+    // the first launch loads both, so that a capture that follows one step outside it loads no code
+    static bool loaded[64][2] = {};
+    if (c->device < 0 || c->device >= 64) return cudaErrorInvalidDevice;
+    if (!loaded[c->device][fused ? 1 : 0]) {
+        cudaFuncAttributes at;
+        const cudaError_t err = cudaFuncGetAttributes(&at, T > 1 ? one : many);
+        if (err != cudaSuccess) return err;
+        loaded[c->device][fused ? 1 : 0] = true;
+    }
     k<<<grid, kAgentWarps * 32, 0, s>>>(a, K);
     return cudaGetLastError();
 }

@@ -728,11 +728,11 @@ k_step_resident(const ResArgs a, const __grid_constant__ RateConsts Kc) {
 
 constexpr int kMaxDev = 64;
 
-// Per-instantiation launch facts, cached per device so that a launch after
-// the first one makes no attribute or occupancy query.
+// Per-instantiation launch facts (CTAs an SM with `smem` bytes), cached per
+// device so that a launch after the first one makes no attribute or occupancy
+// query.
 template <int NT, bool FUSED>
-cudaError_t launch_t(const jwf_ctx* c, const ResArgs& a, const RateConsts& K, size_t smem, cudaStream_t s,
-                     int32_t nq) {
+cudaError_t blocks_t(const jwf_ctx* c, size_t smem, int* blocks) {
     constexpr int kSlots = 8;
     static size_t set_smem[kMaxDev] = {};
     static size_t occ_smem[kMaxDev][kSlots] = {};
@@ -758,11 +758,33 @@ cudaError_t launch_t(const jwf_ctx* c, const ResArgs& a, const RateConsts& K, si
         occ_blocks[dev][slot] = per_sm;
         occ_smem[dev][slot] = smem;
     }
-    if (occ_blocks[dev][slot] < 1) return cudaErrorInvalidConfiguration;
-    int64_t grid = (int64_t)occ_blocks[dev][slot] * c->num_sms;
-    if (grid > nq) grid = nq;
+    *blocks = occ_blocks[dev][slot];
+    return *blocks < 1 ? cudaErrorInvalidConfiguration : cudaSuccess;
+}
+
+template <int NT, bool FUSED>
+cudaError_t launch_t(const jwf_ctx* c, const ResArgs& a, const RateConsts& K, size_t smem, cudaStream_t s,
+                     int32_t nq) {
+    int blocks = 0;
+    const cudaError_t err = blocks_t<NT, FUSED>(c, smem, &blocks);
+    if (err != cudaSuccess) return err;
+    const int64_t grid = std::min<int64_t>((int64_t)blocks * c->num_sms, nq);
     k_step_resident<NT, FUSED><<<(unsigned)grid, NT, smem, s>>>(a, K);
     return cudaGetLastError();
+}
+
+template <bool FUSED>
+cudaError_t blocks_v(const jwf_ctx* c, int threads, size_t smem) {
+    int blocks = 0;
+    switch (threads) {
+        case 32: return blocks_t<32, FUSED>(c, smem, &blocks);
+        case 64: return blocks_t<64, FUSED>(c, smem, &blocks);
+        case 128: return blocks_t<128, FUSED>(c, smem, &blocks);
+        case 256: return blocks_t<256, FUSED>(c, smem, &blocks);
+        case 512: return blocks_t<512, FUSED>(c, smem, &blocks);
+        case 1024: return blocks_t<1024, FUSED>(c, smem, &blocks);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 template <bool FUSED>
@@ -819,6 +841,8 @@ static void res_caps(const jwf_ctx* c, const JwfGroup& G, int threads, int32_t* 
     *qcap = (int32_t)std::max<int64_t>(std::min(want_q, room), kResQMin);
 }
 
+constexpr int32_t kShortLaunch = 4;      // steps below which a launch's grids run about equally long
+
 // Threads for the envs of a size class: as many as one env can use (256 up to
 // 384 words, 512 up to 2048, else 1024) while all envs, spread over the SMs, ask
 // for less than about twice the 1024 threads an SM holds; more envs leave fewer
@@ -840,7 +864,7 @@ static int res_threads(const jwf_ctx* c, const JwfGroup& G, int32_t k) {
                       : words <= 2048 ? 256
                       : words <= 6000 ? 512
                                       : 1024;
-    const int64_t per_sm = (c->flags & JWF_AUTO_RESET) != 0u || k < 4 ? 1024 : 1970;
+    const int64_t per_sm = (c->flags & JWF_AUTO_RESET) != 0u || k < kShortLaunch ? 1024 : 1970;
     while (t > least && (int64_t)t * c->N > per_sm * c->num_sms) t /= 2;
     return t;
 }
@@ -984,6 +1008,19 @@ cudaError_t launch_resident_part(jwf_ctx* c, int32_t k, const int32_t* drops, co
         if (threads != 32 && threads != 64 && threads != 128 && threads != 512 && threads != 1024) threads = 256;
         res_caps(c, G, threads, &a.qcap, &a.lcap);
         const size_t smem = res_smem(G.maxH, G.maxW, a.qcap, a.lcap);
+        if (c->threads_per_env == 0 && G.threads == 0) {
+            // launches of another length may take another block size: its facts
+            // are looked up here too, so that after one step outside a capture
+            // no launch inside it makes a query
+            const int other = res_threads(c, G, k < kShortLaunch ? kShortLaunch : 1);
+            if (other != threads) {
+                int32_t qcap = 0, lcap = 0;
+                res_caps(c, G, other, &qcap, &lcap);
+                const size_t need = res_smem(G.maxH, G.maxW, qcap, lcap);
+                err = fused ? blocks_v<true>(c, other, need) : blocks_v<false>(c, other, need);
+                if (err != cudaSuccess) return err;
+            }
+        }
         cudaStream_t gs = s;
         if (ng > 1) {
             gs = c->side[g];

@@ -45,7 +45,8 @@ class GraphRollout:
         self.graph = None
         if capture:
             # launch once outside capture so that every per-kernel attribute
-            # and occupancy query is cached, then capture
+            # and occupancy query is cached (the library makes those of longer
+            # launches along with the first), then capture
             self._body(1)
             self.prev.zero_()
             torch.cuda.synchronize()
