@@ -6,7 +6,8 @@ Each candidate is timed with CUDA events on a short probe of the caller's own
 workload (the Sim, its initial states and drops); the Sim is restored to the
 initial states afterwards.  Choices are cached in a JSON file (path from the
 JWF_AUTOTUNE_CACHE environment variable, default ~/.cache/jwf_autotune.json),
-keyed by the batch's shape signature, kernel and device name.
+keyed by the batch's shape signature, kernel, device name and the library's
+sources (a choice made for other kernels is not taken over).
 """
 from __future__ import annotations
 
@@ -17,7 +18,7 @@ import os
 import numpy as np
 import torch
 
-from . import jwf
+from . import build, jwf
 
 THREADS = (32, 64, 128, 256, 512, 1024)
 TILE_THREADS = (128, 256, 512)
@@ -58,7 +59,7 @@ def signature(sim: jwf.Sim, kernel: int, probe_steps: int) -> str:
     h.update(shapes.tobytes())
     h.update(counts.tobytes())
     dev = torch.cuda.get_device_name(torch.cuda.current_device())
-    return f"{dev}|k{kernel}|p{probe_steps}|{h.hexdigest()[:20]}"
+    return f"{dev}|k{kernel}|p{probe_steps}|{h.hexdigest()[:20]}|s{build.source_hash()}"
 
 
 def _time(fn, reps: int = 2, prep=None) -> float:

@@ -7,6 +7,7 @@ PyTorch loads, so device pointers and streams pass straight through).
 from __future__ import annotations
 
 import concurrent.futures as cf
+import hashlib
 import os
 import shutil
 import subprocess
@@ -38,6 +39,15 @@ def _deps() -> list[str]:
     files = sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
     files.append(os.path.join(INCLUDE, "jwf.h"))
     return files
+
+
+def source_hash() -> str:
+    """Of the library's sources: what was measured on other kernels has another one."""
+    h = hashlib.sha256()
+    for f in sorted(_deps()):
+        with open(f, "rb") as src:
+            h.update(os.path.basename(f).encode() + b"\0" + hashlib.sha256(src.read()).digest())
+    return h.hexdigest()[:12]
 
 
 def up_to_date() -> bool:
