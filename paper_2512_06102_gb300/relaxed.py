@@ -60,10 +60,22 @@ def theta_to_params(theta: torch.Tensor, n_classes: int, cell_size: float = 30.0
                         mu_veg=np.array(v[6:6 + C], np.float32), mu_den=np.array(v[6 + C:6 + 2 * C], np.float32))
 
 
-def _adjoint_chunk(sim, su, sb, gu, gb, ngu, ngb, masks, scratch, gr, gpc):
-    """Adjoint of one block of steps, its rate adjoint added to gr; scratch [CHUNK or, on chip, 2 * CHUNK, cells]."""
+def _adjoint_scratch(sim, T, masked, device):
+    """(scratch of a backward over T steps, whether its adjoint runs on chip).  The on-chip adjoint takes twice the
+    sweeps' scratch; where the memory left does not hold it, the sweeps run.  (Allocated after everything else.)"""
+    n, cells = min(CHUNK, max(T, 1)), sim.cells
+    if sim.relaxed_on_chip(masked):
+        try:
+            return torch.empty((2 * n, cells), dtype=torch.float32, device=device), True
+        except torch.cuda.OutOfMemoryError:
+            pass
+    return torch.empty((n, cells), dtype=torch.float32, device=device), False
+
+
+def _adjoint_chunk(sim, su, sb, gu, gb, ngu, ngb, masks, scratch, on_chip, gr, gpc):
+    """Adjoint of one block of steps, its rate adjoint added to gr."""
     n = su.shape[0]
-    if sim.relaxed_on_chip(masks is not None):
+    if on_chip:
         sim.relaxed_bwd_rates(su, sb, gu, gb, ngu, ngb, scratch[:2 * n], gr, masks=masks, gpc=gpc)
         return
     sim.relaxed_bwd_steps(su, sb, gu, gb, ngu, ngb, masks=masks, glam=scratch[:n], gpc=gpc)
@@ -130,9 +142,8 @@ class RelaxedRollout(torch.autograd.Function):
             pu_buf = torch.empty((seg, cells), dtype=torch.float32, device=dev)
             pb_buf = torch.empty((seg, cells), dtype=torch.float32, device=dev)
         gr = torch.zeros((cells, 8), dtype=torch.float32, device=dev)     # rate adjoint
-        rows = CHUNK * (2 if sim.relaxed_on_chip(masks is not None) else 1)
-        scratch = torch.empty((rows, cells), dtype=torch.float32, device=dev)
         ngu, ngb = torch.empty_like(gu), torch.empty_like(gb)
+        scratch, on_chip = _adjoint_scratch(sim, T, masks is not None, dev)
         for si in reversed(range(n_seg)):
             a = si * seg
             b = min(a + seg, T)
@@ -153,7 +164,8 @@ class RelaxedRollout(torch.autograd.Function):
             while hi > a:
                 lo = max(a, ((hi - 1) // CHUNK) * CHUNK)
                 mk = None if masks is None else masks[lo:hi]
-                _adjoint_chunk(sim, su[lo - a:hi - a], sb[lo - a:hi - a], gu, gb, ngu, ngb, mk, scratch, gr, gpc)
+                _adjoint_chunk(sim, su[lo - a:hi - a], sb[lo - a:hi - a], gu, gb, ngu, ngb, mk, scratch,
+                               on_chip, gr, gpc)
                 gu, ngu = ngu, gu
                 gb, ngb = ngb, gb
                 hi = lo
@@ -215,13 +227,12 @@ class StraightThroughRollout(torch.autograd.Function):
         gu = (g_un if g_un is not None else torch.zeros(cells, device=dev)).contiguous().clone()
         gb = (g_burn if g_burn is not None else torch.zeros(cells, device=dev)).contiguous().clone()
         ngu, ngb = torch.empty_like(gu), torch.empty_like(gb)
-        rows = CHUNK * (2 if sim.relaxed_on_chip() else 1)
-        scratch = torch.empty((rows, cells), dtype=torch.float32, device=dev)
         gr = torch.zeros((cells, 8), dtype=torch.float32, device=dev)
+        scratch, on_chip = _adjoint_scratch(sim, T, False, dev)
         hi = T
         while hi > 0:
             lo = ((hi - 1) // CHUNK) * CHUNK
-            _adjoint_chunk(sim, PU[lo:hi], PB[lo:hi], gu, gb, ngu, ngb, None, scratch, gr, gpc)
+            _adjoint_chunk(sim, PU[lo:hi], PB[lo:hi], gu, gb, ngu, ngb, None, scratch, on_chip, gr, gpc)
             gu, ngu = ngu, gu
             gb, ngb = ngb, gb
             hi = lo
