@@ -521,8 +521,12 @@ JWF_API jwf_status jwf_relaxed_bwd_steps(jwf_ctx* ctx, int32_t n_steps, const fl
  * added to, d_scratch is float [2][n_steps][cells].  Only where
  * jwf_relaxed_on_chip(ctx, with_masks) is 1 (every grid's rates fit a
  * thread-block cluster's shared memory, and the relaxed kernel is not
- * JWF_RELAXED_PLAIN), else JWF_EUNSUPPORTED. */
+ * JWF_RELAXED_PLAIN), else JWF_EUNSUPPORTED.  jwf_relaxed_on_chip_faster: 1
+ * where that is so and the call is the faster of the two ways, by an estimate;
+ * sparse != 0 where d_pburn is 0 but at the fire fronts (a sampled trajectory).
+ * (Many large grids, of which few fit the GPU at once, are not.) */
 JWF_API int32_t jwf_relaxed_on_chip(jwf_ctx* ctx, int32_t with_masks);
+JWF_API int32_t jwf_relaxed_on_chip_faster(jwf_ctx* ctx, int32_t with_masks, int32_t sparse);
 JWF_API jwf_status jwf_relaxed_bwd_rates(jwf_ctx* ctx, int32_t n_steps, const float* d_pun,
                                          const float* d_pburn, const float* d_masks,
                                          const float* d_gun_out, const float* d_gburn_out, float* d_gun,

@@ -1023,6 +1023,10 @@ int32_t jwf_relaxed_on_chip(jwf_ctx* ctx, int32_t with_masks) {
     return ctx != nullptr && ctx->d_r != nullptr && jwf_band_fits(ctx, true, with_masks != 0) ? 1 : 0;
 }
 
+int32_t jwf_relaxed_on_chip_faster(jwf_ctx* ctx, int32_t with_masks, int32_t sparse) {
+    return jwf_relaxed_on_chip(ctx, with_masks) && jwf_band_pays(ctx, with_masks != 0, sparse != 0) ? 1 : 0;
+}
+
 jwf_status jwf_relaxed_bwd_rates(jwf_ctx* ctx, int32_t n_steps, const float* d_pun, const float* d_pburn,
                                  const float* d_masks, const float* d_gun_out, const float* d_gburn_out,
                                  float* d_gun, float* d_gburn, float* d_scratch, float* d_gr, double* d_gpc,

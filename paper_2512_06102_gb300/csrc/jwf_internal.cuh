@@ -420,8 +420,10 @@ cudaError_t jwf_launch_relaxed_bwd(jwf_ctx* c, const float* pun, const float* pb
 // the relaxed steps with the rates kept on chip over the call (k_band.cu): n
 // steps forward (states after each step out), n steps of the adjoint with
 // dL/dlam [n][cells] and, where p_burn is not 0, the incoming dL/dp_burn
-// [n][cells] out; jwf_band_fits: the context's shapes have a plan
+// [n][cells] out; jwf_band_fits: the context's shapes have a plan; jwf_band_pays:
+// the adjoint is faster than the column sweeps (sparse: p_burn 0 but at the fronts)
 bool jwf_band_fits(jwf_ctx* c, bool bwd, bool masked);
+bool jwf_band_pays(jwf_ctx* c, bool masked, bool sparse);
 cudaError_t jwf_launch_band_fwd(jwf_ctx* c, int32_t n, const float* pun, const float* pburn, const float* masks,
                                 float* pun_out, float* pburn_out, cudaStream_t s);
 cudaError_t jwf_launch_band_bwd(jwf_ctx* c, int32_t n, const float* pun, const float* pburn, const float* masks,

@@ -103,6 +103,7 @@ _SIGS = {
     "jwf_relaxed_fwd_steps": (ctypes.c_int, [_VP, ctypes.c_int32] + [_VP] * 6),
     "jwf_relaxed_bwd_steps": (ctypes.c_int, [_VP, ctypes.c_int32] + [_VP] * 10),
     "jwf_relaxed_on_chip": (ctypes.c_int32, [_VP, ctypes.c_int32]),
+    "jwf_relaxed_on_chip_faster": (ctypes.c_int32, [_VP, ctypes.c_int32, ctypes.c_int32]),
     "jwf_relaxed_bwd_rates": (ctypes.c_int, [_VP, ctypes.c_int32] + [_VP] * 11),
     "jwf_rates_contract": (ctypes.c_int, [_VP] * 8),
     "jwf_mask_words": (ctypes.c_int64, [ctypes.c_int64]),
@@ -593,6 +594,10 @@ class Sim:
     def relaxed_on_chip(self, with_masks: bool = False) -> bool:
         """relaxed_bwd_rates takes this context's grids."""
         return bool(lib().jwf_relaxed_on_chip(self._h, int(bool(with_masks))))
+
+    def relaxed_on_chip_faster(self, with_masks: bool = False, sparse: bool = False) -> bool:
+        """It does, and is the faster way (sparse: p_burn is 0 but at the fire fronts)."""
+        return bool(lib().jwf_relaxed_on_chip_faster(self._h, int(bool(with_masks)), int(bool(sparse))))
 
     def relaxed_bwd_rates(self, pun, pburn, gun_out, gburn_out, gun, gburn, scratch, gr, masks=None, gpc=None,
                           stream=None):

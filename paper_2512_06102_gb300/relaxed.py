@@ -60,11 +60,11 @@ def theta_to_params(theta: torch.Tensor, n_classes: int, cell_size: float = 30.0
                         mu_veg=np.array(v[6:6 + C], np.float32), mu_den=np.array(v[6 + C:6 + 2 * C], np.float32))
 
 
-def _adjoint_scratch(sim, T, masked, device):
+def _adjoint_scratch(sim, T, masked, sparse, device):
     """(scratch of a backward over T steps, whether its adjoint runs on chip).  The on-chip adjoint takes twice the
     sweeps' scratch; where the memory left does not hold it, the sweeps run.  (Allocated after everything else.)"""
     n, cells = min(CHUNK, max(T, 1)), sim.cells
-    if sim.relaxed_on_chip(masked):
+    if sim.relaxed_on_chip_faster(masked, sparse):
         try:
             return torch.empty((2 * n, cells), dtype=torch.float32, device=device), True
         except torch.cuda.OutOfMemoryError:
@@ -143,7 +143,7 @@ class RelaxedRollout(torch.autograd.Function):
             pb_buf = torch.empty((seg, cells), dtype=torch.float32, device=dev)
         gr = torch.zeros((cells, 8), dtype=torch.float32, device=dev)     # rate adjoint
         ngu, ngb = torch.empty_like(gu), torch.empty_like(gb)
-        scratch, on_chip = _adjoint_scratch(sim, T, masks is not None, dev)
+        scratch, on_chip = _adjoint_scratch(sim, T, masks is not None, False, dev)
         for si in reversed(range(n_seg)):
             a = si * seg
             b = min(a + seg, T)
@@ -228,7 +228,7 @@ class StraightThroughRollout(torch.autograd.Function):
         gb = (g_burn if g_burn is not None else torch.zeros(cells, device=dev)).contiguous().clone()
         ngu, ngb = torch.empty_like(gu), torch.empty_like(gb)
         gr = torch.zeros((cells, 8), dtype=torch.float32, device=dev)
-        scratch, on_chip = _adjoint_scratch(sim, T, False, dev)
+        scratch, on_chip = _adjoint_scratch(sim, T, False, True, dev)
         hi = T
         while hi > 0:
             lo = ((hi - 1) // CHUNK) * CHUNK

@@ -1,5 +1,6 @@
-"""The backward passes where device memory holds the column sweeps' scratch but not the on-chip adjoint's: the sweeps run, over
-the same blocks of steps (CPU: a simulator that records its calls, an allocator that refuses the larger tensor)."""
+"""The backward passes where device memory holds the column sweeps' scratch but not the on-chip adjoint's, and where the
+library finds the sweeps faster: the sweeps run, over the same blocks of steps and with their scratch (CPU: a simulator that
+records its calls, an allocator that refuses the larger tensor)."""
 import types
 
 import pytest
@@ -13,11 +14,15 @@ CELLS = 6
 class RecordingSim:
     cells, grad_size, n_classes, tables_version = CELLS, 7, 1, 0
 
-    def __init__(self):
-        self.calls = []
+    def __init__(self, faster=True):
+        self.calls, self.faster, self.asked = [], faster, []
 
     def relaxed_on_chip(self, with_masks=False):
         return True
+
+    def relaxed_on_chip_faster(self, with_masks=False, sparse=False):
+        self.asked.append((with_masks, sparse))
+        return self.faster
 
     def relaxed_bwd_rates(self, su, sb, gu, gb, ngu, ngb, scratch, gr, masks=None, gpc=None):
         self.calls.append(("on chip", su.shape[0], scratch.shape[0]))
@@ -59,3 +64,11 @@ def test_sweeps_where_the_larger_scratch_does_not_fit(kind, monkeypatch):
     sim = RecordingSim()
     _backward(kind, sim, T)
     assert sim.calls == [("sweeps", 4, 4), ("rates", 4, 4), ("sweeps", 16, 16), ("rates", 16, 16)]
+
+
+@pytest.mark.parametrize("kind", [relaxed.RelaxedRollout, relaxed.StraightThroughRollout])
+def test_sweeps_where_they_are_faster(kind):
+    sim = RecordingSim(faster=False)
+    _backward(kind, sim, 20)
+    assert sim.calls == [("sweeps", 4, 4), ("rates", 4, 4), ("sweeps", 16, 16), ("rates", 16, 16)]
+    assert sim.asked == [(False, kind is relaxed.StraightThroughRollout)]
