@@ -329,7 +329,7 @@ typedef enum {
 } jwf_kernel;
 /* Choose the step kernel; threads_per_env = 0 picks a block size by env size
  * and number (resident kernels) or 512 threads a tile, with the table and more
- * than 2048 tiles 256 (tiled kernels); else 32, 64, 128, 256, 512 or 1024
+ * than 4096 tiles 256 (tiled kernels); else 32, 64, 128, 256, 512 or 1024
  * threads per env (resident kernels) or 128, 256 or 512 threads a tile (tiled
  * kernels).  Other values return JWF_EINVAL. */
 JWF_API jwf_status jwf_set_kernel(jwf_ctx* ctx, jwf_kernel kernel, int32_t threads_per_env);

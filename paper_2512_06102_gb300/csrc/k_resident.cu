@@ -845,16 +845,23 @@ constexpr int32_t kShortLaunch = 4;      // steps below which a launch's grids r
 
 // Threads for the envs of a size class: as many as one env can use (256 up to
 // 384 words, 512 up to 2048, else 1024) while all envs, spread over the SMs, ask
-// for less than about twice the 1024 threads an SM holds; more envs leave fewer
-// threads each, down to a floor (an env whose planes fill an SM has it alone).
-// With auto-reset all envs run as long, and in a launch of few steps nearly so:
-// there they should start at once, for a second wave costs as much as the first
-// (647 ragged grids of 32 to 50, 116 steps: 256 threads, 608 at once, 834 us).
-// us, 100 steps: 1 of 64 x 64: 64 threads 584, 256 293; 1200: 128 threads 358,
-// 256 394.  304 of 128 x 128: 128 threads 767, 512 576; 1200: 256 825, 512 1129;
-// 5000: 128 1664, 256 2328.  608 of 300 x 300: 256 2782, 512 1720, 1024 2597.
-// 304 of 512 x 512: 512 4185, 1024 1694.  40 launches of one step of 1000 of 100
-// x 75: 128 1085, 256 1280.
+// for less than 1970 threads an SM, a little below twice the 1024 it holds; more
+// envs leave fewer threads each, down to a floor (an env whose planes fill an SM
+// has it alone).  With auto-reset all envs run as long, and in a launch of few
+// steps nearly so: there they should start at once, for a second wave costs as
+// much as the first (647 ragged grids of 32 to 50, 116 steps: 256 threads, 608 at
+// once, 834 us).
+// The line, us for 100 steps with drops, more and fewer threads, at the grids
+// nearest below and above it: 64 x 64, 1100 (1853 threads an SM at 256): 256 326,
+// 128 303; 1216 (2048): 362, 304.  100 x 75, 1000 (1684): 544, 541; 1216: 550,
+// 574; 1400 (2358): 625, 516.  128 x 128, 540 (1819 at 512): 512 634, 256 674; 608
+// (2048): 672, 653; 850: 842, 759.  200 x 200, 420 (1415): 967, 1089; 540: 1247,
+// 1111; 608: 1299, 1188.  The sides cross between 1200 and 2300; a line at 2048
+// itself would leave 608 grids (four an SM at 512 threads) on the slower side.
+// Few grids: 1 of 64 x 64: 64 threads 584, 256 293.  Many: 5000 of 128 x 128: 128
+// 1664, 256 2328.  The floor: 608 of 300 x 300: 256 2782, 512 1720, 1024 2597; 304
+// of 512 x 512: 512 4185, 1024 1694.  40 launches of one step of 1000 of 100 x
+// 75: 128 1085, 256 1280.
 static int res_threads(const jwf_ctx* c, const JwfGroup& G, int32_t k) {
     const int64_t words = (int64_t)G.maxH * ((G.maxW + 31) / 32);
     int t = words <= 384 ? 256 : words <= 2048 ? 512 : 1024;

@@ -980,10 +980,12 @@ cudaError_t jwf_launch_step_tiled(jwf_ctx* c, int32_t k, const int32_t* drops, c
         a.p_continue = c->P.p_continue;
         // 512 threads a tile: a round is as long as its slowest tile, and few
         // of a map's tiles are active.  With the table, whose items are light,
-        // 256 once many tiles are (us: 4 x 4096^2 fused, 500 steps: 256 threads
-        // 6307, 512 5003; 3 x 1531 x 1117 table, 150 steps: 1436 and 1194; 50 x
-        // 600 x 1200 table, 200 steps: 2431 and 2707).
-        const int nt = c->threads_per_env > 0 ? c->threads_per_env : fused || c->n_tiles4 <= 2048 ? 512 : 256;
+        // 256 once many tiles are.  us, 150 steps with drops, 256 and 512
+        // threads: fused, 10 x 600 x 1200 (1000 tiles) 1710 and 1367, 50 of them
+        // 2023 and 1924; table, 10 of them 1456 and 1188, 30 (3000 tiles) 1585
+        // and 1295, 40 1616 and 1600, 50 1720 and 1793; 2 x 4096^2 (4096 tiles)
+        // 1431 and 1189.
+        const int nt = c->threads_per_env > 0 ? c->threads_per_env : fused || c->n_tiles4 <= 4096 ? 512 : 256;
         if (nt == 128)
             err = fused ? launch_tiled_t<128, true>(c, a, K, s) : launch_tiled_t<128, false>(c, a, K, s);
         else if (nt == 512)
