@@ -668,15 +668,19 @@ def bench_relaxed(args, D, dev, rank):
     ach_f = fwd1_b * cells / k_tiled["fwd"] / 1e9
     ach_f2 = 2 * fwd_b * cells / k_tiled["fwd2"] / 1e9
     rate = D.world * cells * REL_T / t_keep
+    # what the rollout's own kernels move: the rates once a call where they stay on chip
+    path_f, path_fn = (8, "on-chip") if sim.relaxed_on_chip() else (fwd_b, "two-step")
+    path_b, path_bn = (12, "on-chip") if sim.relaxed_on_chip_faster() else (bwd_b, "two-step fused")
+    path = path_f + path_b + acc_b
     sim.close()
     return {"metric": "fwd+bwd cell-steps/s at 256x128^2, T=100",
             "value": rate, "unit": "fwd+bwd cell-steps/s",
             "ms_per_step": t_keep * 1e3, "dtype": "f32", "clocks": clock_rec.get((REL_T, None)),
             "memory_policy": "every state kept" if keep_all == 0 else "sqrt(T) checkpoints",
-            "path_bytes_model": f"{fwd_b + bwd_b + acc_b} B/cell-step ({fwd_b} two-step fwd + {bwd_b} two-step "
-                                f"fused adjoint + {acc_b} rate-adjoint accumulation)",
-            "path_gbs": round((fwd_b + bwd_b + acc_b) * rate / D.world / 1e9, 1),
-            "path_frac": round((fwd_b + bwd_b + acc_b) * rate / D.world / 1e9 / hbm, 4),
+            "path_bytes_model": f"{path} B/cell-step ({path_f} {path_fn} fwd + {path_b} {path_bn} adjoint + "
+                                f"{acc_b} rate-adjoint accumulation)",
+            "path_gbs": round(path * rate / D.world / 1e9, 1),
+            "path_frac": round(path * rate / D.world / 1e9 / hbm, 4),
             "roofline": {"bound": "hbm", "achieved": round(ach_b, 1), "peak": hbm, "unit": "GB/s",
                          "frac": round(ach_b / hbm, 4), "peak_source": peak_kind,
                          "traffic": kernel_traffic("k_relaxed_bwd_sweep2", "paper_2512_06102_gb300/csrc/k_relaxed.cu"),

@@ -384,10 +384,13 @@ JWF_API jwf_status jwf_set_reorder_steps(jwf_ctx* ctx, int32_t steps);
 JWF_API jwf_status jwf_set_env_priority(jwf_ctx* ctx, const float* h_priority);
 
 /* Instrumentation: while d_counts (four uint64 on the device, owned by the
- * caller) is set, the resident step kernels add to them the work they did:
+ * caller) is set, the resident and tiled step kernels add to them the work
+ * they did:
  * [0] (target, burning source) pairs compared (the table reads of the byte
  * model), [1] Philox blocks drawn for can-burn cells, [2] remain-burning
- * draws, [3] 32-cell bit-plane words scanned (one per word per step).
+ * draws, [3] 32-cell bit-plane words scanned (one per word per step, in the
+ * groups of up to 32 words that held any of the other three).  The tiled step's
+ * counts include its halos.
  * NULL switches counting off (the default). */
 JWF_API jwf_status jwf_set_pair_counter(jwf_ctx* ctx, unsigned long long* d_counts);
 
@@ -450,6 +453,10 @@ JWF_API jwf_status jwf_agent_rollout(jwf_ctx* ctx, int32_t n_steps, const int32_
  * thread per cell; the adjoint is two kernels (lam adjoint, then the
  * transpose gather) with a round trip of glam through memory.  lam is summed
  * in the same order by both; the gather's order differs (rounding only).
+ * Calls of several steps take two steps a pass and, with JWF_RELAXED_TILED and
+ * grids whose rates fit a thread-block cluster (about 65,000 cells), the
+ * forward of three steps and more keeps the rates on chip over the call
+ * (jwf_relaxed_bwd_rates does so in the adjoint); the results are the same.
  * Rates whose source lies outside the grid are multiplied by zero (they must
  * be finite; jwf_precompute_probs writes 0 there). */
 enum jwf_relaxed_kernel { JWF_RELAXED_TILED = 0, JWF_RELAXED_PLAIN = 1 };
@@ -495,8 +502,8 @@ JWF_API jwf_status jwf_rates_bwd(jwf_ctx* ctx, int32_t n_steps, const float* d_g
                          const float* d_dem, const float* d_wind_speed,
                          const float* d_wind_dir, double* d_gparams, void* stream);
 
-/* n_steps relaxed steps in one call (one kernel launch per step, no host
- * work in between).  Forward: d_pun_out / d_pburn_out are [n_steps][cells],
+/* n_steps relaxed steps in one call (one kernel launch where the rates stay
+ * on chip, else one per two steps; no host work in between).  Forward: d_pun_out / d_pburn_out are [n_steps][cells],
  * row t the state after step t, which starts from row t - 1 (from d_pun /
  * d_pburn for t = 0); d_masks is [n_steps][cells] or NULL.  The outputs must
  * not overlap the inputs.  Same requirements as jwf_step_relaxed_fwd. */

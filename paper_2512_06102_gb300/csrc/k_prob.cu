@@ -1,12 +1,13 @@
 // k_prob.cu -- per-(cell, direction) ignition tables (Section 3, Eqs. 1-4)
 // and their parameter gradient.
 //
-// k_prob_table: one thread per target cell v computes, for the 8 incoming
-// directions d (source u = v - Delta_d),
+// k_prob_table: for a target cell v and the 8 incoming directions d (source u =
+// v - Delta_d),
 //   r[v][d] = gamma(v) * phi(u, d),   q[v][d] = 1 - exp(-r[v][d])
 // with phi from Eq. 3 (wind Eq. 1 and slope Eq. 2 taken at the source) and
-// gamma the target's susceptibility.  HBM-write bound: 32 B of q (and 32 B of
-// r) per cell against 5 B of class + elevation read.
+// gamma the target's susceptibility.  A CTA takes a tile of cells: the slope part
+// once for each edge between two cells, then a thread a cell.  Bound by FP32
+// issue (75% active), not by the 32 B of q (and 32 B of r) a cell.
 //
 // k_rates_bwd: dL/dtheta = sum_t sum_{v,d} glam_t(v) pb_t(v - Delta_d) dr[v][d]/dtheta,
 // every derivative written without division so that classes with no fuel
