@@ -58,3 +58,25 @@ def test_few_large_grids_are_tiled(H, W, many, same_as):
     assert torch.equal(state[jwf.KERNEL_FUSED], state[jwf.KERNEL_TILED_FUSED])
     equal = work[jwf.KERNEL_FUSED] == work[jwf.KERNEL_TILED_FUSED]
     assert equal == (same_as is not None)
+
+
+def test_few_large_grids_with_auto_reset():
+    """The automatic choice steps them one step a launch on the plain kernel and several on the resident one, in turn."""
+    require_gpu()
+    scn = scenarios.make_scenario(617, 641, N=2, seed=5)
+    sim = make_sim(scn, seed=3, auto_reset=True, t_max=5)
+    sim.precompute_probs(*[to(a) for a in (scn.cls, scn.dem, scn.wind_speed, scn.wind_dir)])
+    q = sim.probs()[0].cpu().numpy().copy()
+    sim.load_state(to(scn.F0))
+    drops = scenarios.drops(12, scn.H, scn.W, seed=2, p_drop=0.5)
+    outs, t = [], 0
+    for k in (1, 3, 1, 1, 6):
+        outs.append([x.cpu().numpy() for x in sim.step(k, to(drops[t:t + k]))])
+        t += k
+    state = sim.state().cpu().numpy()
+    sim.close()
+    ro = discrete.Rollout(scn.H, scn.W, scn.F0, q, scn.params.p_continue, seed=3, t_max=5, auto_reset=True)
+    want = ro.step(12, drops)
+    np.testing.assert_array_equal(state, ro.F)
+    for i in range(3):
+        np.testing.assert_array_equal(np.concatenate([o[i] for o in outs]), want[i])
